@@ -21,12 +21,21 @@ namespace {
 __device__ __forceinline__ float4 ld4g(const float* p) { return *reinterpret_cast<const float4*>(p); }
 constexpr float4 ZERO4 = {0.f, 0.f, 0.f, 0.f};
 
+// c + alpha v of every term the element has, rounded term by term: the same bits as one launch a term
+template <int TERMS>
+__device__ __forceinline__ float add_terms(float c, float alpha, const float (&v)[TERMS], const bool (&has)[TERMS]) {
+#pragma unroll
+    for (int q = 0; q < TERMS; ++q)
+        if (has[q]) c = c + alpha * v[q];
+    return c;
+}
+
 // ---------------------------------------------------------------- N <= 4
 // Warp = R rows of A; lanes over K, U float4 a lane and row in flight.  triA: 1 lower, 2 upper triangular.
 template <int TERMS, int R, int U, int NB>
-__global__ void __launch_bounds__(256) rows_nt_kernel(int M, int N, int K, float alpha, ProdTerms P, int64_t lda,
-                                                      int64_t sA, int64_t ldb, int64_t sB, float beta, float* C,
-                                                      int64_t ldc, int64_t sC, int transC, int triA) {
+__global__ void __launch_bounds__(256, TERMS) rows_nt_kernel(int M, int N, int K, float alpha, ProdTerms P, int64_t lda,
+                                                             int64_t sA, int64_t ldb, int64_t sB, float beta, float* C,
+                                                             int64_t ldc, int64_t sC, int transC, int triA) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row0 = (blockIdx.x * 8 + warp) * R, bt = blockIdx.y;
     C += (int64_t)bt * sC;
@@ -34,11 +43,13 @@ __global__ void __launch_bounds__(256) rows_nt_kernel(int M, int N, int K, float
     int k0 = 0, k1 = K;
     if (triA == 1) k1 = min(K, (last + 4) & ~3);
     if (triA == 2) k0 = min(row0, M - 1) & ~3;
-    float acc[R][NB];
+    float acc[TERMS][R][NB];                                   // a sum per term: C takes them one after another
 #pragma unroll
-    for (int r = 0; r < R; ++r)
+    for (int q = 0; q < TERMS; ++q)
 #pragma unroll
-        for (int n = 0; n < NB; ++n) acc[r][n] = 0.f;
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int n = 0; n < NB; ++n) acc[q][r][n] = 0.f;
     bool has[TERMS];                                           // (one term: every element has it)
 #pragma unroll
     for (int q = 0; q < TERMS; ++q) has[q] = TERMS == 1 || (bt >= P.lo[q] && bt < P.hi[q]);
@@ -77,7 +88,8 @@ __global__ void __launch_bounds__(256) rows_nt_kernel(int M, int N, int K, float
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         const float4 v = a[term][r][u];
-                        acc[r][n] = fmaf(v.x, b.x, fmaf(v.y, b.y, fmaf(v.z, b.z, fmaf(v.w, b.w, acc[r][n]))));
+                        float& s = acc[term][r][n];
+                        s = fmaf(v.x, b.x, fmaf(v.y, b.y, fmaf(v.z, b.z, fmaf(v.w, b.w, s))));
                     }
                 }
             }
@@ -87,13 +99,17 @@ __global__ void __launch_bounds__(256) rows_nt_kernel(int M, int N, int K, float
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
-            float v = acc[r][n];
+            float v[TERMS];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            for (int q = 0; q < TERMS; ++q) {
+                v[q] = acc[q][r][n];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+            }
             const int row = row0 + r;
             if (lane == n && n < N && row < M) {
                 float* c = transC ? C + (int64_t)n * ldc + row : C + (int64_t)row * ldc + n;
-                *c = (beta == 0.f ? 0.f : beta * *c) + alpha * v;
+                *c = add_terms<TERMS>(beta == 0.f ? 0.f : beta * *c, alpha, v, has);
             }
         }
 }
