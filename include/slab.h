@@ -164,7 +164,9 @@ slab_status slab_factor(const slab_grid* grid, const slab_coeffs* coeffs, int b,
  * Solve A u = f for k right-hand sides (Algorithm 4 + iterative refinement).
  * f, u: device, [k][(n-1)^d]; u is overwritten.  relres_out: HOST, k entries
  * (may be NULL) receiving ||f - A u||_2/||f||_2; iters_out: HOST (may be NULL)
- * receiving the number of refinement steps taken.  Returns SLAB_ENOCONV when
+ * receiving the number of refinement steps taken.  Refinement ends at the first residual with
+ * max_k relres <= rtol: the error of u is then what that residual leaves, up to the conditioning
+ * times rtol, and a smaller rtol asks for less.  Returns SLAB_ENOCONV when
  * max_refine steps did not reach rtol, when the residual stagnated (two steps without halving
  * the worst relative residual), or when it is not finite (relres_out then holds NaN); u holds
  * the last iterate.
