@@ -166,7 +166,10 @@ slab_status slab_factor(const slab_grid* grid, const slab_coeffs* coeffs, int b,
  * (may be NULL) receiving ||f - A u||_2/||f||_2; iters_out: HOST (may be NULL)
  * receiving the number of refinement steps taken.  Refinement ends at the first residual with
  * max_k relres <= rtol: the error of u is then what that residual leaves, up to the conditioning
- * times rtol, and a smaller rtol asks for less.  Returns SLAB_ENOCONV when
+ * times rtol, and a smaller rtol asks for less.  HELMHOLTZ and CONVECTION (krylov 0), whose residual
+ * says less about the error, take one more step where that residual lies above rtol / 10, the step
+ * before gained at least a factor 100 and max_refine allows it; u is the iterate with the smaller
+ * residual, so the tolerance stays met (a copy of u is held meanwhile).  Returns SLAB_ENOCONV when
  * max_refine steps did not reach rtol, when the residual stagnated (two steps without halving
  * the worst relative residual), or when it is not finite (relres_out then holds NaN); u holds
  * the last iterate.
