@@ -217,14 +217,6 @@ __global__ void __launch_bounds__(256) gemm_tn_skinny_kernel(int M, int N, int K
 // Bound by the chain of its 16 steps: in FP32 the two barriers, the 4 x 4 factor and the shared-memory round trips
 // (four entries an access; a panel pair with two of these tiles 34.5 -> 30.4 us), in FP64 by the
 // multiply-adds, one per sub-partition every 64 cycles (137 -> 125 us; the blocks packed into whole warps).
-// The tile's reciprocal root.  FP32 keeps the form r (1.5 - a r^2 / 2), whose error is below two units in the last
-// place: with rsqrt_newton the residual after a refinement pass of a 3-D solve is 0.87 of this one's (n = 35, b = 7,
-// 3 loads: 8.6e-11 and 9.9e-11), which ends solves near the tolerance a pass sooner.
-__device__ __forceinline__ float rsqrt_tile(float a) {
-    const float r = rsqrtf(a);
-    return r * (1.5f - 0.5f * a * r * r);
-}
-__device__ __forceinline__ double rsqrt_tile(double a) { return rsqrt_newton(a); }
 // A usable Cholesky pivot: positive and finite (NaN fails both comparisons), in T's own arithmetic.
 __device__ __forceinline__ bool pivot_ok(float d) { return d > 0.0f && d <= 3.402823466e38f; }
 __device__ __forceinline__ bool pivot_ok(double d) { return d > 0.0 && d <= 1.7976931348623157e308; }
@@ -1031,12 +1023,6 @@ struct GeppSmem {
     int go;
 };
 
-// 1 / x to FP32 rounding: the hardware's approximation and one Newton step (x normal, below 2^126).
-__device__ __forceinline__ float reciprocal(float x) {
-    const float r = __fdividef(1.f, x);
-    return fmaf(r, fmaf(-x, r, 1.f), r);
-}
-
 // Partial-pivoting elimination of up to ROWS rows x 64 columns, thread t holding row t in registers
 // (have: it holds one), in blocks of 8 columns.  In a block, each of the 8 steps has one barrier: every
 // warp publishes its best row's 8 columns, and after the barrier every thread picks the best warp (first
@@ -1084,7 +1070,7 @@ __device__ __forceinline__ void gj_gepp(float (&a)[64], bool have, GeppSmem<ROWS
                 mine = jj;
                 sm.order[jb + jj] = t;
             }
-            const float l = bk > 1u ? a[jj] * reciprocal(p[jj]) : 0.f;   // a pivot that is not zero
+            const float l = bk > 1u ? pivot_quotient(a[jj], p[jj], bk - 1u) : 0.f;   // a pivot that is not zero
             lm[jj] = l;
             if (emit) {
                 const bool ok = bk > 1u && bk <= 0x7f800000u;            // and finite

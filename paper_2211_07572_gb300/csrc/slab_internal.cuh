@@ -418,18 +418,15 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // the rounding error has no preferred sign: pivots too small throughout by one part in 10^7 shift the
 // operator's spectrum by that times its largest eigenvalue, which an FP32 factor of a fine grid feels.
 // (n = 2048, b = 32: each refinement pass gains a factor 70, and four reach 1e-10; with r (1.5 - a r^2 / 2) the
-// same solve needed more passes.)  FP64: two steps from the hardware's approximation (about 2^-20 -> 2^-39 ->
-// rounding), in fewer of the slow FP64 instructions than the library's function.
+// same solve needed more passes.)  FP64: two steps from the hardware's approximation (about 2^-20 -> 2^-39 -> within one
+// unit in the last place), in fewer of the slow FP64 instructions than the library's function.
 __device__ __forceinline__ float rsqrt_newton(float a) {
     const float r = rsqrtf(a);
     return fmaf(0.5f * r, fmaf(-a * r, r, 1.0f), r);
 }
 __device__ __forceinline__ double rsqrt_newton(double a) {
     const unsigned hi = (unsigned)__double2hiint(a);
-    if (hi < 0x01000000u || hi >= 0x7e000000u) {               // tiny, huge, negative or NaN
-        const double r = rsqrt(a);
-        return r * (1.5 - 0.5 * a * r * r);
-    }
+    if (hi < 0x01000000u || hi >= 0x7e000000u) return rsqrt(a);   // tiny (half of a may underflow), huge, negative or NaN
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
 #pragma unroll
@@ -437,9 +434,18 @@ __device__ __forceinline__ double rsqrt_newton(double a) {
     return r;
 }
 
+// The reciprocal root of the 64 x 64 Cholesky tiles (dense.cu).  FP32 keeps the form r (1.5 - a r^2 / 2), whose error is below two units in the last
+// place: with rsqrt_newton the residual after a refinement pass of a 3-D solve is 0.87 of this one's (n = 35, b = 7,
+// 3 loads: 8.6e-11 and 9.9e-11), which ends solves near the tolerance a pass sooner.
+__device__ __forceinline__ float rsqrt_tile(float a) {
+    const float r = rsqrtf(a);
+    return r * (1.5f - 0.5f * a * r * r);
+}
+__device__ __forceinline__ double rsqrt_tile(double a) { return rsqrt_newton(a); }
+
 // 1 / x, x finite and not zero.  FP64: two Newton steps r <- r + r (1 - x r) from the hardware's approximation
-// (about 2^-20 -> 2^-40 -> rounding) where the exponent leaves room for them: four of the slow FP64
-// instructions in place of a division's chain.
+// (about 2^-20 -> 2^-40 -> within one unit in the last place) where the exponent leaves room for them: four of the slow
+// FP64 instructions in place of a division's chain.
 __device__ __forceinline__ float reciprocal_full(float x) { return 1.0f / x; }
 __device__ __forceinline__ double reciprocal_full(double x) {
     const unsigned mag = (unsigned)__double2hiint(x) & 0x7fffffffu;
@@ -449,6 +455,20 @@ __device__ __forceinline__ double reciprocal_full(double x) {
 #pragma unroll
     for (int it = 0; it < 2; ++it) r = fma(r, fma(-x, r, 1.0), r);
     return r;
+}
+
+// 1 / x within one unit in the last place: the hardware's approximation and one Newton step.  x normal and below 2^126
+// (beyond, the approximation is zero).
+__device__ __forceinline__ float reciprocal(float x) {
+    const float r = __fdividef(1.f, x);
+    return fmaf(r, fmaf(-x, r, 1.f), r);
+}
+// a / p, |a| <= |p|, for a finite pivot p whose magnitude's bits are mag (known before p is, in a pivot search).  Both are
+// scaled by a power of two where the reciprocal of p is not a normal number (the multipliers of a pivot above 2^126
+// were zero otherwise, unflagged).
+__device__ __forceinline__ float pivot_quotient(float a, float p, unsigned mag) {
+    const float s = mag >= 0x7e800000u ? 0.25f : (mag < 0x00800000u ? 4294967296.f : 1.f);
+    return (a * s) * reciprocal(p * s);
 }
 
 // error helper: latches SLAB_ECUDA in the handle; with SLAB_CUDA_TRACE set in the environment it
