@@ -34,7 +34,8 @@
  *     by the caller.  With k == 0 right-hand sides a call does nothing and
  *     its vector pointers may be NULL.  Calls are asynchronous on opts.stream except where a
  *     host output is requested; those synchronise that stream before return.
- *   - The handle owns all factor memory; release it with slab_destroy().
+ *   - The handle owns all factor memory; release it with slab_destroy().  The library keeps part of what
+ *     closed handles held, for the next one (slab_release_memory).
  *   - No C++ exception crosses the ABI.  Errors are returned as slab_status;
  *     the first CUDA error is also latched in the handle (slab_last_error).
  *   - A handle may be used by one host thread at a time.
@@ -393,6 +394,16 @@ int64_t slab_device_bytes(const slab_handle* h);
 slab_status slab_last_error(const slab_handle* h);
 
 void slab_destroy(slab_handle* h);
+
+/*
+ * Device memory of handles comes from a pool of the library's own, one per device, which keeps up to a
+ * sixth of the device's memory after handles are closed: a factor allocates and frees about 40 buffers,
+ * and mapping them anew costs about 1 ms per GB.  The library gives all of it back by itself where one
+ * of its own allocations (a handle, a batch, slab_tc_gemm) would fail otherwise; other allocators in the
+ * process cannot ask for it.  This call returns what the current device's pool holds unused, except
+ * keep_bytes of it, to the device.  Waits for the device's work.  SLAB_EINVAL for keep_bytes < 0.
+ */
+slab_status slab_release_memory(int64_t keep_bytes);
 const char* slab_strerror(slab_status s);
 
 /*

@@ -62,6 +62,7 @@ SIGNATURES = {
     "slab_stage2_order": (c_int, [c_void_p]),
     "slab_last_error": (c_int, [c_void_p]),
     "slab_destroy": (None, [c_void_p]),
+    "slab_release_memory": (c_int, [c_int64]),
     "slab_strerror": (ctypes.c_char_p, [c_int]),
     "slab_profile": (c_int, [c_void_p, c_int]),
     "slab_profile_read": (c_int, [c_void_p, c_void_p, c_void_p, c_int]),

@@ -287,7 +287,12 @@ slab_status slab_batch_create(int count, const int* n, const int* b, const slab_
     if (st) { slab_batch_destroy(B); return st; }
     const size_t io_bytes = (io.off + 255) & ~(size_t)255;
     B->bytes = io_bytes + wave_max;
-    if (cudaMalloc(&B->mem, B->bytes) != cudaSuccess) {
+    cudaError_t e = cudaMalloc(&B->mem, B->bytes);
+    if (e != cudaSuccess) {                            // handles closed before may have left memory in the pool
+        cudaGetLastError();
+        if (slab_give_back(nullptr)) e = cudaMalloc(&B->mem, B->bytes);
+    }
+    if (e != cudaSuccess) {
         cudaGetLastError();
         B->mem = nullptr;
         slab_batch_destroy(B);

@@ -222,6 +222,9 @@ inline bool sizing_pass(const slab_handle* h) { return h->arena && !h->arena->ba
 // Device allocation of a handle's buffer (from its arena if it has one; counted in dev_bytes).
 slab_status slab_dalloc(slab_handle* h, void** p, size_t bytes);
 void slab_dfree(slab_handle* h, void* p);
+// Give back what the device pool holds unused, before an allocation outside it is tried once more.  Does nothing (false)
+// while st is under capture.
+bool slab_give_back(cudaStream_t st);
 // slab_factor in steps: create validates and allocates every buffer the factor needs (no kernel
 // runs); launch enqueues the factor on h->stream with no allocation and no host synchronisation;
 // factor_status synchronises the stream and maps the device status word to a slab_status.

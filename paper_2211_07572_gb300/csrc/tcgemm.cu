@@ -1292,7 +1292,12 @@ extern "C" slab_status slab_tc_gemm(int M, int N, int K, float alpha, const floa
     if (K <= 0 || K % 64) return SLAB_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     g.w16_bytes = f16x3_work_bytes(M, N, K, 1, f16x3_shared(g));
-    if (cudaMallocAsync(&g.w16, g.w16_bytes, st) != cudaSuccess) {
+    cudaError_t e = cudaMallocAsync(&g.w16, g.w16_bytes, st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        if (slab_give_back(st)) e = cudaMallocAsync(&g.w16, g.w16_bytes, st);
+    }
+    if (e != cudaSuccess) {
         cudaGetLastError();
         return SLAB_ENOMEM;
     }

@@ -32,6 +32,13 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
+def release_memory(keep_bytes: int = 0, device=None):
+    """Return the device memory that the library keeps from closed solvers, except keep_bytes of it, to the device
+    (slab_release_memory).  Waits for the device's work."""
+    with torch.cuda.device(torch.device("cuda" if device is None else device)):
+        _lib.check(_lib.load().slab_release_memory(int(keep_bytes)), "slab_release_memory")
+
+
 class SlabSolver:
     """Factor A for one grid/coefficient set (Algorithm 3) and solve with it (Algorithm 4).
 
