@@ -396,9 +396,11 @@ slab_status slab_last_error(const slab_handle* h);
 void slab_destroy(slab_handle* h);
 
 /*
- * Device memory of handles comes from a pool of the library's own, one per device, which keeps up to a
- * sixth of the device's memory after handles are closed: a factor allocates and frees about 40 buffers,
- * and mapping them anew costs about 1 ms per GB.  The library gives all of it back by itself where one
+ * Device memory of handles comes from a pool of the library's own, one per device, which keeps memory
+ * after handles are closed: a factor allocates and frees about 40 buffers, and mapping them anew costs
+ * about 1 ms per GB.  It keeps about what was in use together at most since no handle was open the last time
+ * (less use lowers that by a quarter each time the last handle closes), and never more than a quarter
+ * of the device's memory.  The library gives all of it back by itself where one
  * of its own allocations (a handle, a batch, slab_tc_gemm) would fail otherwise; other allocators in the
  * process cannot ask for it.  This call returns what the current device's pool holds unused, except
  * keep_bytes of it, to the device.  Waits for the device's work.  SLAB_EINVAL for keep_bytes < 0.

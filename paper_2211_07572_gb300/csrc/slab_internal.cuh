@@ -160,7 +160,7 @@ struct slab_handle {
     size_t red_cap, ticket_cap;
 
     int64_t dev_bytes;
-    void* unpooled;           // std::vector<void*>: buffers allocated outside the device pool (during a capture)
+    void* bufs;               // std::vector<Buffer> (api.cu): the handle's buffers, with their sizes and pools
     slab_status err;
 
     // measurement: launch counts per kernel class, optional event timing

@@ -67,3 +67,30 @@ def test_an_allocation_that_needs_the_kept_memory(what):
         del ballast
         torch.cuda.empty_cache()
         release_memory()
+
+
+def test_what_is_kept_follows_use():
+    """One large handle, then small ones: each round with no handle left lowers the kept memory by a quarter.  (3/4)^13 of 13 GiB
+    is 0.3 GiB; the driver's pieces and the small handles make up the rest of the bound."""
+    release_memory()
+    before = _free()
+    held = _close_a_handle()
+    kept = before - _free()
+    assert held // 2 <= kept <= held + held // 4 + GIB // 4
+    for _ in range(13):
+        s = SlabSolver(2, 128, 16, inputs.POISSON, precision="fp32")
+        s.close()
+        torch.cuda.synchronize()
+    assert before - _free() <= GIB
+    release_memory()
+
+
+def test_never_more_than_a_quarter_of_the_device_is_kept():
+    release_memory()
+    before = _free()
+    s = SlabSolver(2, 4096, 32, inputs.POISSON, precision="fp32", stage2="oddeven")
+    total = torch.cuda.mem_get_info()[1]
+    assert s.device_bytes > total // 3
+    s.close()
+    assert total // 8 <= before - _free() <= total // 4 + GIB // 4
+    release_memory()
