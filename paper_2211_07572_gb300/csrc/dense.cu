@@ -865,7 +865,7 @@ slab_status launch_fp64_product(slab_handle* h, int M, int N, int K, double alph
                                 int64_t ldc, int64_t sC, int transC, int lower_only, int batch, int mcut, int ncut) {
     if (M <= 0 || N <= 0) return SLAB_OK;
     const dim3 big((N + TL - 1) / TL, (M + TL - 1) / TL, batch);
-    if ((int64_t)big.x * big.y * batch < 4 * 152 && (M + 15) / 16 <= 65535)
+    if ((int64_t)big.x * big.y * batch < 4 * SMS && (M + 15) / 16 <= 65535)
         SLAB_CK(h, launch_pdl(gemm_tn_spread_kernel<double>, dim3((N + 15) / 16, (M + 15) / 16, batch), dim3(256), 0,
                               h->stream, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, transC, lower_only, sA, sB, sC,
                               mcut, ncut));
@@ -1696,7 +1696,7 @@ __global__ void convert_kernel(const S* __restrict__ src, D* __restrict__ dst, i
 slab_status widen_to_double(slab_handle* h, const float* src, double* dst, int64_t n) {
     if (n <= 0) return SLAB_OK;
     SLAB_PROF(h, KC_OTHER);
-    convert_kernel<float, double><<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 16), 256, 0, h->stream>>>(
+    convert_kernel<float, double><<<(unsigned)std::min<int64_t>((n + 255) / 256, SMS * 16), 256, 0, h->stream>>>(
         src, dst, n);
     SLAB_CK_LAUNCH(h);
     return SLAB_OK;
@@ -1705,7 +1705,7 @@ slab_status widen_to_double(slab_handle* h, const float* src, double* dst, int64
 slab_status narrow_to_float(slab_handle* h, const double* src, float* dst, int64_t n) {
     if (n <= 0) return SLAB_OK;
     SLAB_PROF(h, KC_OTHER);
-    convert_kernel<double, float><<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 16), 256, 0, h->stream>>>(
+    convert_kernel<double, float><<<(unsigned)std::min<int64_t>((n + 255) / 256, SMS * 16), 256, 0, h->stream>>>(
         src, dst, n);
     SLAB_CK_LAUNCH(h);
     return SLAB_OK;
@@ -2203,7 +2203,7 @@ slab_status tall_update(slab_handle* h, T* W, int ncols, int rows, int c0, int c
 // on the 152 SMs (two CTAs per SM): then every CTA can factor the diagonal tile itself and the separate
 // diagonal launch is saved.  FP64 panels factor it once and spread everything else over the SMs: the
 // fused kernels' redundant products cost 65 us each there (n = 128, b = 16 Poisson solve 6.5 -> 3.7 ms).
-inline bool one_wave(int64_t ctas) { return ctas <= 2 * 152; }
+inline bool one_wave(int64_t ctas) { return ctas <= 2 * SMS; }
 
 template <typename T>
 slab_status tall_panel(slab_handle* h, T* W, int ncols, int ident0, int kb, int batch, int64_t bstride, size_t smem) {
@@ -2294,7 +2294,7 @@ slab_status tall_chol_range(slab_handle* h, T* W, int ncols, int ident0, int kb0
     // fill the GPU anyway, and there its redundant tile products cost more than the launches it saves
     const int64_t tiles = (int64_t)batch * ((ident0 + (kb0 + 1) * TL) / TL - kb0 - 1);
     if constexpr (sizeof(T) == 4)
-        if (kb1 - kb0 == 2 && tiles <= 8 * 152) return tall_pair<T>(h, W, ncols, ident0, kb0, batch, bstride, smem);
+        if (kb1 - kb0 == 2 && tiles <= 8 * SMS) return tall_pair<T>(h, W, ncols, ident0, kb0, batch, bstride, smem);
     const int kbm = kb0 + (kb1 - kb0) / 2;
     slab_status st;
     if ((st = tall_chol_range<T>(h, W, ncols, ident0, kb0, kbm, batch, bstride, smem))) return st;

@@ -226,12 +226,14 @@ void slab_dfree(slab_handle* h, void* p);
 // while st is under capture.
 bool slab_give_back(cudaStream_t st);
 // slab_factor in steps: create validates and allocates every buffer the factor needs (no kernel
-// runs); launch enqueues the factor on h->stream with no allocation and no host synchronisation;
+// runs; in three dimensions all but Stage 2's); launch enqueues the factor on h->stream, in two dimensions with no
+// allocation and no host synchronisation (three: alloc_stage2 between the stages);
 // factor_status synchronises the stream and maps the device status word to a slab_status.
 slab_status factor_create(const slab_grid* grid, const slab_coeffs* co, int b, const slab_opts* opts,
                           slab_handle** out, SlabArena* arena);
 slab_status factor_launch(slab_handle* h, const double* kappa, const double* c);
 slab_status factor_status(slab_handle* h);
+slab_status alloc_stage2(slab_handle* h);
 // Every buffer a solve of k loads needs (solve workspace, FP64 residual, norm reduction).
 slab_status solve_prepare(slab_handle* h, int k);
 // Zero the self-resetting ticket counters of a handle whose memory may hold another's old data.
@@ -473,6 +475,8 @@ __device__ __forceinline__ float pivot_quotient(float a, float p, unsigned mag) 
     const float s = mag >= 0x7e800000u ? 0.25f : (mag < 0x00800000u ? 4294967296.f : 1.f);
     return (a * s) * reciprocal(p * s);
 }
+
+constexpr int SMS = 152;   // of a GB300: the wave that dispatch rules on grid sizes count with
 
 // error helper: latches SLAB_ECUDA in the handle; with SLAB_CUDA_TRACE set in the environment it
 // also prints the CUDA error and the source line of the failed call (run with

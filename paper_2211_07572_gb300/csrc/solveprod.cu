@@ -262,11 +262,11 @@ static slab_status launch_products(slab_handle* h, int M, int N, int K, float al
     };
     const int64_t rows = (int64_t)M * batch;
     cudaError_t e;
-    if (N == 1) e = rows >= 32 * 4 * 152 ? go(rows_nt_kernel<TERMS, 4, 2, 1>, 32) : go(rows_nt_kernel<TERMS, 1, 8, 1>, 8);
-    else if (N <= 4) e = rows >= 32 * 4 * 152 ? go(rows_nt_kernel<TERMS, 4, 2, 4>, 32) : go(rows_nt_kernel<TERMS, 1, 8, 4>, 8);
-    else if (N <= 8) e = rows >= 32 * 2 * 152 ? go(stream_nt_kernel<TERMS, 2, 1>, 32) : go(stream_nt_kernel<TERMS, 1, 1>, 16);
-    else if (N <= 16) e = rows >= 32 * 2 * 152 ? go(stream_nt_kernel<TERMS, 2, 2>, 32) : go(stream_nt_kernel<TERMS, 1, 2>, 16);
-    else if (TERMS == 1 && rows >= 32 * 2 * 152) e = go(stream_nt_kernel<1, 2, 4>, 32);
+    if (N == 1) e = rows >= 32 * 4 * SMS ? go(rows_nt_kernel<TERMS, 4, 2, 1>, 32) : go(rows_nt_kernel<TERMS, 1, 8, 1>, 8);
+    else if (N <= 4) e = rows >= 32 * 4 * SMS ? go(rows_nt_kernel<TERMS, 4, 2, 4>, 32) : go(rows_nt_kernel<TERMS, 1, 8, 4>, 8);
+    else if (N <= 8) e = rows >= 32 * 2 * SMS ? go(stream_nt_kernel<TERMS, 2, 1>, 32) : go(stream_nt_kernel<TERMS, 1, 1>, 16);
+    else if (N <= 16) e = rows >= 32 * 2 * SMS ? go(stream_nt_kernel<TERMS, 2, 2>, 32) : go(stream_nt_kernel<TERMS, 1, 2>, 16);
+    else if (TERMS == 1 && rows >= 32 * 2 * SMS) e = go(stream_nt_kernel<1, 2, 4>, 32);
     else e = go(stream_nt_kernel<TERMS, 1, 4>, 16);
     SLAB_CK(h, e);
     return SLAB_OK;

@@ -197,7 +197,7 @@ struct StencilGrid {
         const int s = n - 1, gx = (s + 255) / 256;
         q = k == 1 ? 1 : (k <= 4 ? 4 : ST_Q);
         const int gz = (k + q - 1) / q;
-        rows = (int64_t)gx * ((s + ST_ROWS - 1) / ST_ROWS) * gz < 2 * 152 ? ST_FEW : ST_ROWS;
+        rows = (int64_t)gx * ((s + ST_ROWS - 1) / ST_ROWS) * gz < 2 * SMS ? ST_FEW : ST_ROWS;
         grid = dim3(gx, (s + rows - 1) / rows, gz);
     }
     template <typename F> void dispatch(F&& f) const {
@@ -547,7 +547,7 @@ slab_status launch_gather_interface(slab_handle* h, const double* v, double* out
     const int64_t tot = (int64_t)k * h->td.NI * h->td.si;
     if (tot <= 0) return SLAB_OK;
     SLAB_PROF(h, KC_OTHER);
-    gather_interface_kernel<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 152 * 32), 256, 0, h->stream>>>(
+    gather_interface_kernel<<<(unsigned)std::min<int64_t>((tot + 255) / 256, SMS * 32), 256, 0, h->stream>>>(
         h->dim, h->n, h->b, h->td.NI, k, v, out);
     SLAB_CK_LAUNCH(h);
     return SLAB_OK;
@@ -574,14 +574,14 @@ slab_status vec_dot(slab_handle* h, const double* x, const double* y, int64_t N,
 
 slab_status vec_axpy(slab_handle* h, double* y, const double* x, const double* c, double sign, int64_t N, int k) {
     SLAB_PROF(h, KC_OTHER);
-    vaxpy_kernel<<<dim3(2 * 152, k), 256, 0, h->stream>>>(y, x, c, sign, N);
+    vaxpy_kernel<<<dim3(2 * SMS, k), 256, 0, h->stream>>>(y, x, c, sign, N);
     SLAB_CK_LAUNCH(h);
     return SLAB_OK;
 }
 
 slab_status vec_scale(slab_handle* h, double* x, const double* nrm2, int64_t N, int k) {
     SLAB_PROF(h, KC_OTHER);
-    vscale_kernel<<<dim3(2 * 152, k), 256, 0, h->stream>>>(x, nrm2, N);
+    vscale_kernel<<<dim3(2 * SMS, k), 256, 0, h->stream>>>(x, nrm2, N);
     SLAB_CK_LAUNCH(h);
     return SLAB_OK;
 }
@@ -589,7 +589,7 @@ slab_status vec_scale(slab_handle* h, double* x, const double* nrm2, int64_t N, 
 slab_status vec_combine(slab_handle* h, double* u, const double* Z, int64_t zstride, const double* c, int j, int k,
                         int64_t N) {
     SLAB_PROF(h, KC_OTHER);
-    vcombine_kernel<<<dim3(2 * 152, k), 256, 0, h->stream>>>(u, Z, zstride, c, j, k, N);
+    vcombine_kernel<<<dim3(2 * SMS, k), 256, 0, h->stream>>>(u, Z, zstride, c, j, k, N);
     SLAB_CK_LAUNCH(h);
     return SLAB_OK;
 }

@@ -1235,7 +1235,8 @@ slab_status tc_gemm(cudaStream_t st, TcGemmArgs& g, unsigned* err) {
         if (narrow) return launch_f16x3<64>(st, g, err);
         return f16x3_use_wide(g) ? launch_f16x3<256>(st, g, err) : launch_f16x3<128>(st, g, err);
     }
-    // few right-hand sides (the solve products): 32-wide tiles leave room for a fifth stage in flight
+    // few columns (slab_tc_gemm, and solve products whose operands the streaming kernels cannot take): 32-wide tiles leave
+    // room for a fifth stage in flight
     if (g.split && g.N <= 32) return launch_tc<32, true>(st, g, err);
     if (g.split && !narrow && g.K <= 2 * BK) return launch_tc<64, true, true>(st, g, err);
     if (g.split) return narrow ? launch_tc<64, true>(st, g, err) : launch_tc<128, true>(st, g, err);

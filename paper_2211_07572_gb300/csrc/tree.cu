@@ -31,9 +31,7 @@ __device__ __forceinline__ void lds4(const double* p, double (&v)[4]) {
 }
 __device__ __forceinline__ bool usable_square(float d) { return d > 0.0f && d <= 3.402823466e38f; }
 __device__ __forceinline__ bool usable_square(double d) { return d > 0.0 && d <= 1.7976931348623157e308; }
-__device__ __forceinline__ unsigned magnitude(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 __device__ __forceinline__ unsigned magnitude(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
-__device__ __forceinline__ bool usable_magnitude(float v) { return magnitude(v) != 0u && magnitude(v) < 0x7f800000u; }
 __device__ __forceinline__ bool usable_magnitude(double v) {
     return (magnitude(v) | (unsigned)__double2loint(v)) != 0u && magnitude(v) < 0x7ff00000u;
 }

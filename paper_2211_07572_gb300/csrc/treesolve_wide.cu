@@ -320,7 +320,7 @@ constexpr int DCW_MIN = 32;
 // enough CTAs to fill the GPU (about 4 per SM) without chunks narrower than DCW_MIN.
 inline int down_chunk(int nodes, int wmax) {
     int c = DCW;
-    while (c > DCW_MIN && (int64_t)nodes * ((2 * wmax + c - 1) / c) < 4 * 152) c /= 2;
+    while (c > DCW_MIN && (int64_t)nodes * ((2 * wmax + c - 1) / c) < 4 * SMS) c /= 2;
     return c;
 }
 template <typename T, bool INDEF>
