@@ -1309,10 +1309,9 @@ extern "C" slab_status slab_tc_gemm(int M, int N, int K, float alpha, const floa
 
 // C (FP64, M x N, ldc) += alpha A B^T with A (M x K, lda) and B (N x K, ldb) FP64, FP64-accurate
 // on the tensor cores (integer-slice products, above).  K <= 64, K % 32 == 0.  work: FP16
-// slices [OZ_S][M][K] and [OZ_S][N][K] followed by the exponents (M + N ints): ozaki_work_bytes (which
-// leaves room for 32-bit slices).
+// slices [OZ_S][M][K] and [OZ_S][N][K] followed by the exponents (M + N ints): ozaki_work_bytes.
 size_t ozaki_work_bytes(int64_t M, int64_t N, int K) {
-    return (size_t)OZ_S * (M + N) * K * sizeof(float) + (size_t)(M + N) * sizeof(int) + 256;
+    return (size_t)OZ_S * (M + N) * K * sizeof(__half) + (size_t)(M + N) * sizeof(int) + 256;
 }
 
 slab_status ozaki_gemm(cudaStream_t st, int M, int N, int K, double alpha, const double* A, int64_t lda,
