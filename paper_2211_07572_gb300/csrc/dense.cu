@@ -942,7 +942,7 @@ slab_status gemm_tn<double>(slab_handle* h, int cls, int M, int N, int K, double
 //   G[all, rest] -= G[all, panel] X       (tensor-core rank-64 update of all rows).
 // The s_pad / 64 panel steps of an interface are a serial chain, so their latency is what counts:
 // three launches a step (tournament, which also delivers the LU of A11 in FP32, solve, update).  Measured:
-// convection n = 768, b = 24 factor + solve + adjoint 230 -> 42 ms, Helmholtz n = 512, b = 32 (FP64) 103 -> 28 ms
+// convection n = 768, b = 24 factor + solve + adjoint 230 -> 43 ms, Helmholtz n = 512, b = 32 (FP64) 103 -> 28 ms
 // against one warp per 128-row group in shared memory, LU and solve with barriers every column, and two updates.
 constexpr int GJ_LEAF = 256;          // rows per tournament group, one per thread
 constexpr int GJ_WAY = 4;             // winner sets per merge: GJ_WAY * 64 = GJ_LEAF rows

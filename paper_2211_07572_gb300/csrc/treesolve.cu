@@ -20,7 +20,7 @@
 // lane = row of the separator, the loads in registers, the other operand broadcast.
 //   Measured (FP32, n = 1024, b = 32, one load, kernel times of a pass): up 0.76 -> 0.16 ms, down 0.67 ->
 // 0.19 ms against the kernels of treesolve_wide.cu, which compute 64 loads whatever their number; the low
-// launches run at 52 / 40 % of the HBM peak.  Up to SOLVE_NARROW = 8 loads (n = 777, 5 loads: up + down
+// launches move 4.1 / 3.0 TB/s through DRAM, 61 / 45 % of a plain copy's rate.  Up to SOLVE_NARROW = 8 loads (n = 777, 5 loads: up + down
 // 2.7 -> 0.9 ms a pass) a thread holds them all in registers; beyond, the wide kernels' blocks are fuller.
 #include <algorithm>
 #include <atomic>
