@@ -32,10 +32,14 @@ __device__ __forceinline__ float add_terms(float c, float alpha, const float (&v
 
 // ---------------------------------------------------------------- N <= 4
 // Warp = R rows of A; lanes over K, U float4 a lane and row in flight.  triA: 1 lower, 2 upper triangular.
+//   rows_ctas: CTAs that share an SM, whose loads in flight hide each other's latency.  Without the bound one term and
+// four loads take 222 registers, one CTA; two terms with U = 8 spill.  Two refinement passes: 3-D n = 64, b = 8, 4 loads 5.39 ms,
+// 6.19 without the bounds and with U = 8; n = 35, b = 7, 3 loads 1.71 and 2.09 ms.
+constexpr int rows_ctas(int terms, int nb) { return terms == 2 ? 2 : (nb == 1 ? 4 : 3); }
 template <int TERMS, int R, int U, int NB>
-__global__ void __launch_bounds__(256, TERMS) rows_nt_kernel(int M, int N, int K, float alpha, ProdTerms P, int64_t lda,
-                                                             int64_t sA, int64_t ldb, int64_t sB, float beta, float* C,
-                                                             int64_t ldc, int64_t sC, int transC, int triA) {
+__global__ void __launch_bounds__(256, rows_ctas(TERMS, NB))
+    rows_nt_kernel(int M, int N, int K, float alpha, ProdTerms P, int64_t lda, int64_t sA, int64_t ldb, int64_t sB,
+                   float beta, float* C, int64_t ldc, int64_t sC, int transC, int triA) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row0 = (blockIdx.x * 8 + warp) * R, bt = blockIdx.y;
     C += (int64_t)bt * sC;
@@ -263,7 +267,9 @@ static slab_status launch_products(slab_handle* h, int M, int N, int K, float al
     const int64_t rows = (int64_t)M * batch;
     cudaError_t e;
     if (N == 1) e = rows >= 32 * 4 * SMS ? go(rows_nt_kernel<TERMS, 4, 2, 1>, 32) : go(rows_nt_kernel<TERMS, 1, 8, 1>, 8);
-    else if (N <= 4) e = rows >= 32 * 4 * SMS ? go(rows_nt_kernel<TERMS, 4, 2, 4>, 32) : go(rows_nt_kernel<TERMS, 1, 8, 4>, 8);
+    else if (N <= 4)
+        e = rows >= 32 * 4 * SMS ? go(rows_nt_kernel<TERMS, 4, 2, 4>, 32)
+                                 : go(rows_nt_kernel<TERMS, 1, TERMS == 2 ? 4 : 8, 4>, 8);
     else if (N <= 8) e = rows >= 32 * 2 * SMS ? go(stream_nt_kernel<TERMS, 2, 1>, 32) : go(stream_nt_kernel<TERMS, 1, 1>, 16);
     else if (N <= 16) e = rows >= 32 * 2 * SMS ? go(stream_nt_kernel<TERMS, 2, 2>, 32) : go(stream_nt_kernel<TERMS, 1, 2>, 16);
     else if (TERMS == 1 && rows >= 32 * 2 * SMS) e = go(stream_nt_kernel<1, 2, 4>, 32);
