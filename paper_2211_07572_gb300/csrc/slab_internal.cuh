@@ -115,13 +115,13 @@ struct slab_handle {
     void* tZtb;               // [NS][s+1][m*2m]  Z = Linv B for the top/bot rows
     void* tRtb;               // [NS][s+1][2m*2m] condensed top/bot x top/bot block
     void* tZI;                // [NS][H][2][m][s_pad]  Z for interface nodes, per height
-    void* tRI;                // [NS][H][2][2][m][s_pad] condensed top/bot x interface rows
+    void* tRI;                // [NS][H][2][2][m][s_pad] condensed top/bot x interface rows (factor only)
     void* tWtb;               // Helmholtz only: [NS][s+1][m*2m] W = S^{-1} B (top/bot columns)
     void* tWI;                // Helmholtz only: [NS][H][2][m][s_pad] W for the interface columns
     void* ToT;                // Helmholtz only: [NI-1][s_pad][s_pad] T_{q+1,q} (row-major)
     // CONVECTION only: the elimination of A^T from the same tree (see tree.cu), and Stage 2's
     // T_{q+1,q} plus the transposed factors of the A^T sweep
-    void *tZD, *tZDT;         // [NS][H][2][s_pad][m] ZI (general kinds: WI; tZDT: WIT) node-major
+    void *tZD, *tZDT;         // [NS][H][2][s_pad][m] ZI (general kinds: WI; tZDT: WIT) node-major: the two halves of tRI
     void *tLinvT, *tZtbT, *tWtbT, *tZIT, *tWIT, *tRIc;
     void* Tl;                 // [NI-1][s_pad][s_pad] T_{q+1,q} as assembled (Stage-2 scalar)
     void* Tl1;                // mixed mode: T_{q+1,q} in the Stage-1 scalar (factor only)
